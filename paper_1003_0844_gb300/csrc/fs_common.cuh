@@ -109,7 +109,9 @@ __device__ __forceinline__ float df_mul_frac(df32 a, df32 b) {
 // before has completed and its writes are visible; every kernel launched this way calls
 // it in every thread before it reads or writes anything that an earlier kernel touches,
 // so the order of a whole chain holds.  It does nothing in a kernel launched the ordinary
-// way.  (Letting the next kernel start while blocks of the one before are still at work,
+// way.  Its pointers are not declared __restrict__: the data they point to may still change
+// when such a kernel starts, and the qualifier's promise that it does not would let a load
+// take the read-only path or move above the wait.  (Letting the next kernel start while blocks of the one before are still at work,
 // griddepcontrol.launch_dependents, measured no faster on a search of one template and
 // 40% slower on a segment load, whose waiting blocks then sit beside the working ones:
 // 148.6 us without, 209 us with it, 164 us with ordinary launches.)

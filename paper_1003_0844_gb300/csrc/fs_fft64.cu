@@ -30,8 +30,8 @@ __device__ inline double2 tw_get(const double2 *tw, int64_t e, int64_t half, int
   return w;
 }
 
-__global__ void k_stockham64_r2(const double2 *__restrict__ x, double2 *__restrict__ y,
-                                const double2 *__restrict__ tw, int64_t n, int log2p, int sign, int batch) {
+__global__ void k_stockham64_r2(const double2 *x, double2 *y, const double2 *tw, int64_t n, int log2p, int sign,
+                                int batch) {
   pdl_wait();
   const int64_t h = n >> 1;
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -48,8 +48,8 @@ __global__ void k_stockham64_r2(const double2 *__restrict__ x, double2 *__restri
   ys[j + p] = make_double2(u0.x - u1.x, u0.y - u1.y);
 }
 
-__global__ void k_stockham64_r4(const double2 *__restrict__ x, double2 *__restrict__ y,
-                                const double2 *__restrict__ tw, int64_t n, int log2p, int sign, int batch) {
+__global__ void k_stockham64_r4(const double2 *x, double2 *y, const double2 *tw, int64_t n, int log2p, int sign,
+                                int batch) {
   pdl_wait();
   const int64_t q4 = n >> 2, h = n >> 1;
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -109,9 +109,8 @@ __constant__ double2 kW16[10] = {
 // (c the first DFT's output), 4-point DFTs over b; output index c + 4 d.  (Four
 // lanes per DFT with an exchange through shared memory measured no faster on a
 // single transform and 9% slower on the batched transforms of the FP64 form.)
-__global__ void __launch_bounds__(128) k_stockham64_r16(const double2 *__restrict__ x, double2 *__restrict__ y,
-                                                        const double2 *__restrict__ tw, int64_t n, int log2p, int sign,
-                                                        int batch) {
+__global__ void __launch_bounds__(128) k_stockham64_r16(const double2 *x, double2 *y, const double2 *tw, int64_t n,
+                                                        int log2p, int sign, int batch) {
   pdl_wait();
   const int64_t q16 = n >> 4, h = n >> 1;
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;

@@ -90,10 +90,8 @@ struct PtLayout {
 // t_k = k dt: n0 . r_k and the derivatives of n0 dotted with r_k) instead of the
 // analytic orbit and rotation terms; the sidereal angle still comes from etab.
 template <bool HESS, bool MET, bool EPH>
-__global__ void __launch_bounds__(kPtThreads) k_points(SegGeom g, const dbl4 *__restrict__ etab,
-                                                       const dbl4 *__restrict__ eph,
-                                                       const double *__restrict__ x, const PointConst *pcs,
-                                                       double *partial) {
+__global__ void __launch_bounds__(kPtThreads) k_points(SegGeom g, const dbl4 *etab, const dbl4 *eph,
+                                                       const double *x, const PointConst *pcs, double *partial) {
   pdl_wait();
   using Lt = PtLayout<HESS, MET>;
   constexpr int NA = Lt::kN;
@@ -326,7 +324,7 @@ __device__ __forceinline__ void fast_reduce(const df32 *acc, int q0, int NA, dou
 
 // F and its gradient: accumulators [0, 26) of PtLayout (Sa, Sb, dSa_i, dSb_i, sums of
 // a^2, b^2 and a da, b db).  NA: stride of a block's partials.
-__global__ void __launch_bounds__(kPtThreads) k_points_fg(SegGeom g, const dbl4 *__restrict__ etab, Etab32 et,
+__global__ void __launch_bounds__(kPtThreads) k_points_fg(SegGeom g, const dbl4 *etab, Etab32 et,
                                                           const FastConst *fcs, double *partial, int NA) {
   pdl_wait();
   __shared__ FastConst c;
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(kPtThreads) k_points_fg(SegGeom g, const dbl4 
 // One kernel per signal (SIG 0: a, 1: b), 23 sums each: 2% faster than one kernel with
 // all 46 (255 registers and spills); forcing 3 CTAs per SM (168 registers) gained nothing.
 template <int SIG>
-__global__ void __launch_bounds__(kPtThreads) k_points_h(SegGeom g, const dbl4 *__restrict__ etab, Etab32 et,
+__global__ void __launch_bounds__(kPtThreads) k_points_h(SegGeom g, const dbl4 *etab, Etab32 et,
                                                          const FastConst *fcs, double *partial, int NA, int q0) {
   pdl_wait();
   __shared__ FastConst c;
@@ -385,7 +383,7 @@ namespace fs {
 // The metric's accumulators [26, 40) in FP64 (first pass of a climb only): sums of
 // dP_i and dP_i dP_j [cycles],
 // over every sample, or (nv.nn > 0) over the nodes with their weights.
-__global__ void __launch_bounds__(kPtThreads) k_points_met(SegGeom g, const dbl4 *__restrict__ etab, NodeTab nv,
+__global__ void __launch_bounds__(kPtThreads) k_points_met(SegGeom g, const dbl4 *etab, NodeTab nv,
                                                            const PointConst *pcs, double *partial, int NA) {
   pdl_wait();
   __shared__ PointConst c;

@@ -219,7 +219,7 @@ __host__ __device__ __forceinline__ void sample_geometry(const FastConst &c, df3
 // reaches ~2.5e5 cycles: it is formed in FP64 and reduced to a fraction of a cycle
 // before the rest of the phase is added in double-float (the Hessian's terms cancel to
 // ~1e-4 near a maximum, so both kernels need the same accuracy).
-__host__ __device__ __forceinline__ FastSample fast_sample(const FastConst &c, const SegGeom &g, const dbl4 *__restrict__ etab,
+__host__ __device__ __forceinline__ FastSample fast_sample(const FastConst &c, const SegGeom &g, const dbl4 *etab,
                                                   const Etab32 &et, const float4 *sc, int64_t k) {
   FastSample s;
   const dbl4 e4 = etab[k];

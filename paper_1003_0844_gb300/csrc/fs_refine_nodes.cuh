@@ -256,8 +256,8 @@ struct MomShared {
 // S_3 to S_5 enter below 1e-5 of the result and are FP32.  A point per lane makes the data,
 // the place s and its powers the same for the whole warp (broadcast reads), and leaves
 // nothing to reduce across lanes.
-__global__ void __launch_bounds__(kMomThreads, 4) k_moments(SegGeom g, NodeTab v, const float2 *__restrict__ X,
-                                                         const FastConst *__restrict__ fcs, int npt, float2 *W) {
+__global__ void __launch_bounds__(kMomThreads, 4) k_moments(SegGeom g, NodeTab v, const float2 *X,
+                                                         const FastConst *fcs, int npt, float2 *W) {
   extern __shared__ __align__(16) unsigned char mom_smem[];
   MomShared &S = *(MomShared *)mom_smem;
   float4 *sx = (float4 *)(mom_smem + sizeof(MomShared));  // (x.hi, x.lo, s, sigma^3) per sample
