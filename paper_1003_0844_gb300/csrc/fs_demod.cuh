@@ -56,6 +56,30 @@ inline int dem_block(double dt) {
   return k;
 }
 
+// Spline interval *i and position *f in it of the data at t_j = j dt - phi, that is 2 j - v
+// half-samples with v = phi (2/dt); false outside the data's 2 n - 1 half-samples.
+// FP32 holds v's whole part as far as it matters: an interval of the data has
+// |2 j - v| <= 2 n with j < n <= 2^20, so |v| <= 2^21, where v.hi has two fractional bits and
+// kf +- 1 is exact.  From |v| = 2^24 on (sampling intervals below 6e-5 s, whose whole series
+// is shorter than the delay) kf may miss by whole steps and f leave [0, 1), but t_j then lies
+// |v| - 2^21 half-samples outside and neither is used.  The difference is taken modulo 2^32
+// and compared unsigned: a kf that saturates (|v| >= 2^31, below 5e-7 s) stays outside.
+__host__ __device__ __forceinline__ bool spline_place(df32 phi, df32 two_over_dt, int j, int n, unsigned *i, float *f) {
+  const df32 v = df_mul(phi, two_over_dt);
+  float kf = ceilf(v.hi), fr = (kf - v.hi) - v.lo;
+  if (fr < 0.f) { fr += 1.f; kf += 1.f; }
+  if (fr >= 1.f) { fr -= 1.f; kf -= 1.f; }
+#ifdef __CUDA_ARCH__
+  const int k = __float2int_rz(kf);
+#else
+  const int k = kf >= 2147483648.f ? INT32_MAX : kf <= -2147483648.f ? INT32_MIN : (int)kf;
+#endif
+  const unsigned last = 2u * (unsigned)n - 2u;
+  *i = 2u * (unsigned)j - (unsigned)k;
+  *f = fr;
+  return *i < last || (*i == last && fr == 0.f);
+}
+
 // Steps 1-6 and 8 of one output sample j < n (t_b = j dt):
 //  t_j = m1 dt + tau (one Newton step on t + phi_m(t) = t_b from a first delay
 //  estimate), phi_m(t_j) and its time derivative, x~(t_j), a(t_j), b(t_j) and

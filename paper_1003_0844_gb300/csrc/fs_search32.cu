@@ -442,14 +442,10 @@ __global__ void __launch_bounds__(256) k_demod_poly(DemodArgs A) {
       const df32 phi = quick_two_sum(ps.hi, ps.lo + (f0.y + (fmaf(f0.z, u, -p) + fmaf(f0.w, u, hi))));
       const float av = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, ab.y, ab.x), a0.w), a0.z), a0.y), a0.x);
       const float bv = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, b1.w, b1.z), b1.y), b1.x), ab.w), ab.z);
-      // the data at t_j = j dt - phi: spline interval 2 j - k, position f in it
-      const df32 v = df_mul(phi, A.two_over_dt2);
-      float kf = ceilf(v.hi), f = (kf - v.hi) - v.lo;
-      if (f < 0.f) { f += 1.f; kf += 1.f; }
-      if (f >= 1.f) { f -= 1.f; kf -= 1.f; }
-      const int i = 2 * j - (int)kf, ilast = 2 * n - 2;
+      unsigned i;
+      float f;
       float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-      if ((i >= 0 && i < ilast) || (i == ilast && f == 0.f)) c = A.coef[i];
+      if (spline_place(phi, A.two_over_dt2, j, n, &i, &f)) c = A.coef[i];
       const float xr = fmaf(f, fmaf(f, fmaf(f, c.w, c.z), c.y), c.x);
       const float2 e = expm2pi(df_mul_frac(A.fl, phi));  // heterodyne
       const df32 tau = df_mul_f(A.dt2, (float)j);        // exact index

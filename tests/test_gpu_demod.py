@@ -77,3 +77,35 @@ def test_fp64_transform_of_every_length(fs, p, how):
         assert np.max(np.abs(F[m] - ref) / np.maximum(ref, 1.0)) <= F64_TOL
     sky, spin, k, Fc = res.candidates()
     assert len(k) == np.count_nonzero(F > 12.0) and np.allclose(F[spin, k], Fc, rtol=1e-6)
+
+
+# The delay is up to 4e7 (1e8) half-samples here; the data holds sources whose delay stays
+# within its 2.5 s (1 s), and reads nothing for the others.
+@pytest.mark.parametrize("dt,n", [(2.5e-5, 100001), (1e-5, 100001)])
+def test_short_sampling_intervals_match_oracle(fs, dt, n):
+    """Bounds as at the other intervals (an error of 1e-12 s of the delay is 2e-7 half-samples
+    at most), and the rounding of a and b themselves, sums of five FP32 terms of order one
+    (2.4e-7): they are constant over so short a span, so it does not average out.  A source perpendicular to the Earth's position, one turned from there by a
+    delay of 0.3 of the span (either way), and one whose delay exceeds the span."""
+    det = W.Detector(lambda_e0=1.0)
+    x = np.random.default_rng(n).standard_normal(n).astype(np.float32).astype(np.float64)
+    ctx = fs.Context(det)
+    seg = fs.Segment(ctx, _dev(x, torch.float32), dt, 1 << 17, 435.1875, 2 * dt)
+    oseg = ors.Segment(x, dt)
+    ce, se = np.cos(det.eps), np.sin(det.eps)
+    for lon, lat in ((1.0 + np.pi / 2, 0.8), (1.0 + np.pi / 2 + 0.3 * n * dt / 499.0, 0.1),
+                     (1.0 + np.pi / 2 - 0.3 * n * dt / 499.0, -0.1), (2.0, -0.5)):
+        ec = np.array([np.cos(lat) * np.cos(lon), np.cos(lat) * np.sin(lon), np.sin(lat)])
+        eq = np.array([ec[0], ce * ec[1] - se * ec[2], se * ec[1] + ce * ec[2]])
+        alpha, delta = float(np.arctan2(eq[1], eq[0])), float(np.arcsin(eq[2]))
+        ya, yb, ts, ab = fs.demodulate(ctx, seg, alpha, delta)
+        assert ctx.sync_status() == 0
+        ref = ofs.demodulate(oseg, alpha, delta, 0.0, 435.1875, det)
+        assert np.max(np.abs(ts.cpu().numpy() - ref.t_src)) < 1e-9
+        far = lon == 2.0
+        assert far == (np.count_nonzero(ref.ya) == 0) and (far or np.count_nonzero(ref.ya) > n // 2)
+        for got, want in ((ya, ref.ya), (yb, ref.yb)):
+            assert np.max(np.abs(got.cpu().numpy() - want)) <= 2.4e-6 * np.max(np.abs(want)) + 2.4e-7 * np.max(np.abs(x)) * (not far)
+        a2, b2 = ab.cpu().numpy()
+        for got, want in ((a2, ref.a2), (b2, ref.b2)):
+            assert abs(got / want - 1) < 1e-6 + 4.8e-7 / np.sqrt(want)
