@@ -17,7 +17,7 @@
 // quotient rule.  Four forms: FP64 over every sample for a caller's position table
 // (k_points); with the analytic Earth double-float sums over a few nodes per block of
 // samples (fs_refine_nodes.cuh), or over every sample where the sampling interval is too
-// long for that (k_points_fg, k_points_h).
+// long or the series too short for that (k_points_fg, k_points_h).
 //
 // The hill climb is Newton's method on F with the analytic Hessian (second
 // derivatives from the same pass), damped Levenberg-Marquardt style where F is
@@ -649,8 +649,9 @@ static fs_status alloc_table(void **p, size_t bytes) {
 }
 
 // Samples per sub-block of the sums over nodes, or 0: a caller's position table (its
-// linear pieces are no polynomial) and sampling intervals above 16 s take every sample.
-static int seg_node_sub(const fs_seg *seg) { return seg->eph ? 0 : node_sub(seg->g.dt); }
+// linear pieces are no polynomial), short series and sampling intervals above 16 s take
+// every sample.
+static int seg_node_sub(const fs_seg *seg) { return seg->eph ? 0 : node_sub(seg->g.dt, seg->g.n); }
 
 static fs_status earth_table(fs_seg *seg, cudaStream_t st) {
   const unsigned nb = (unsigned)((seg->g.n + 255) / 256);
@@ -709,8 +710,11 @@ struct RefWs {
   float4 *W;
   int chunk;
 };
-// W takes at most this much (at least 32 points' worth); more points go in turns.
+// W takes at most this much (at least 32 points' worth); more points go in turns.  A point
+// has kNodes kNodeBlocks nodes at least, 3 KB, so a turn holds at most 87,381 points and
+// k_moments' grid 2,731 groups of them in y, whose limit is 65,535.
 constexpr size_t kNodeBytes = (size_t)256 << 20;
+static_assert(kNodeBytes / (sizeof(float4) * kNodes * kNodeBlocks) / 32 < 65535, "groups of points in a grid's y");
 
 static fs_status refine_ws(fs_ctx *ctx, const fs_seg *seg, int npt, bool climb, cudaStream_t st, RefWs *w) {
   int nsm = 0;

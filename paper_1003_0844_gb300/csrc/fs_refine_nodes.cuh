@@ -14,7 +14,11 @@
 // run over 6 nodes per block (one node for 43 samples at dt = 2 s) with W_q in the place
 // of x_k exp(-2 pi i Phi_k).  The error of the interpolation is below
 // (2 Omega_r 256 s)^6 / (6! 2^5) = 1.2e-13 of g's scale (products with a second harmonic of
-// the day; the third and fourth have amplitudes below 1e-4 of it).
+// the day; the third and fourth have amplitudes below 1e-4 of it).  The derivatives with
+// f1 hold t^2, and f1's second one t^4, beside a and b: over a block of length h a series of
+// length T bends these by (h/T)^2 and (h/T)^3 of their scale, times
+// 15 (2 Omega_r 256 s)^4 / (6! 2^5) = 1.2e-9, so a series is cut into 32 blocks at least
+// (node_sub).
 //
 // The phase is needed at every sample, but it too is a polynomial on the block, through
 // its values at the same nodes: (f0 + fl) times the diurnal delay's sixth-order term is
@@ -22,9 +26,12 @@
 // rates, the small rest is interpolated, and the phase then advances from sample to sample
 // by two 64-bit integer additions (units of 2^-64 cycles: reduction modulo 1 is free).
 //
-// Accuracy (single points of half a day to 6 days against sums in 128-bit arithmetic):
-// F 5e-13 .. 1e-11, its gradient 1e-13 .. 2e-11; over every sample it was F 5e-13 .. 5e-11,
-// gradient 2e-12 .. 6e-10, bound by the FP64 phase of each sample (3e-11 cycles).
+// Accuracy (19 lengths from 1024 samples to 6 days at 0.5 to 16 s, against sums in 64-bit
+// mantissas, worst of four points each): F 4e-14 .. 2e-11, the gradient 3e-14 .. 4e-11 and the
+// Hessian 1e-13 .. 1e-11 of F times the phase derivatives that meet in them; over every
+// sample it is F 1e-11 .. 3e-10, gradient 4e-12 .. 3e-10, Hessian 2e-12 .. 1e-9, bound by the
+// FP64 phase of each sample (3e-11 cycles).  With blocks of 512 s whatever the length (one of
+// 256 samples for a series of 200) the gradient was off by up to 1e-8, the Hessian by 3e-7.
 // Measured, 256 points of a 2-day series at 2 s with gradient and Hessian: 4.72 ms over every
 // sample, 0.27 ms this way, about half of it k_moments and half the sums over nodes.
 #pragma once
@@ -35,13 +42,19 @@ constexpr int kNodes = 6;     // nodes per block
 constexpr int kNodeSub = 8;   // sub-blocks per block, one warp each in k_moments
 constexpr int kNodeSubMin = 4, kNodeSubMax = 128;  // samples per sub-block
 
-// Samples per sub-block for a sampling interval: the largest power of two within 64 s, at
-// most 128.  0 (the sums run over every sample): dt above 16 s, where a block would hold
-// no more than five samples per node and the interpolation no longer pays.
-static int node_sub(double dt) {
-  if (!(dt <= 16.0)) return 0;
+// Blocks a series is cut into at least.  The derivatives with f1 hold t^2 and t^4 beside a
+// and b, whose curvature over a block is the larger the fewer blocks there are.
+constexpr int kNodeBlocks = 32;
+
+// Samples per sub-block for a sampling interval and a length: the largest power of two
+// within 64 s, at most 128, that leaves kNodeBlocks blocks.  0 (the sums run over every
+// sample): dt above 16 s, where a block would hold no more than five samples per node and
+// the interpolation no longer pays, and series below kNodeBlocks of the smallest blocks,
+// 1024 samples.
+static int node_sub(double dt, int64_t n) {
+  if (!(dt <= 16.0) || n < (int64_t)kNodeBlocks * kNodeSub * kNodeSubMin) return 0;
   int sb = kNodeSubMin;
-  while (2 * sb <= kNodeSubMax && 2 * sb * dt <= 64.0) sb *= 2;
+  while (2 * sb <= kNodeSubMax && 2 * sb * dt <= 64.0 && n >= (int64_t)kNodeBlocks * kNodeSub * 2 * sb) sb *= 2;
   return sb;
 }
 
@@ -253,7 +266,8 @@ struct MomShared {
 // 68) and a dozen integer instructions for the phase, against ~3500 for the 72 sums
 // themselves.  The real and the imaginary part go through packed pairs: 288 -> 274 us for a
 // step on 256 points (k_moments itself 140 us with scalar instructions, issue 0.65 busy).
-// S_3 to S_5 enter below 1e-5 of the result and are FP32.  A point per lane makes the data,
+// S_3 to S_5 enter with g's third and higher powers over a block, below 2e-5 of the result
+// with 32 blocks, and are FP32.  A point per lane makes the data,
 // the place s and its powers the same for the whole warp (broadcast reads), and leaves
 // nothing to reduce across lanes.
 __global__ void __launch_bounds__(kMomThreads, 4) k_moments(SegGeom g, NodeTab v, const float2 *X,
