@@ -118,6 +118,7 @@ struct fs_seg {
   // and the data as double-floats (same call)
   void *nodes = nullptr;
   float2 *xdf = nullptr;
+  bool nodes_ready = false, etab64_ready = false, etab32_ready = false;  // (not while only recorded in a graph)
   // caller's position table (fs_prepare_segment_eph), else NULL:
   //   eph[2m] = (r_m, 0), eph[2m + 1] = (v_m, 0), m < n (light-seconds, SSB ecliptic frame)
   fs::dbl4 *eph = nullptr;

@@ -642,10 +642,21 @@ __global__ void k_climb_out(int npt, const ClimbState *st, double *F) {
 // The fine search's tables: built by the first call on a segment; the double-float
 // copy of the data is refreshed by every call (fs_seg_load may have replaced it).
 static fs_status alloc_table(void **p, size_t bytes) {
-  if (cudaMalloc(p, bytes) == cudaSuccess) return FS_OK;
+  if (*p || cudaMalloc(p, bytes) == cudaSuccess) return FS_OK;
   cudaGetLastError();
   *p = nullptr;
   return FS_ERR_NOMEM;
+}
+
+// After a table's launch: an error of the launch, or whether later calls may take the table
+// as there.  They may not while the launch is only recorded into a graph, which may be
+// replayed late or never; until a call builds it directly, each builds it for itself.
+static fs_status table_launched(cudaStream_t st, bool *ready) {
+  if (cudaGetLastError() != cudaSuccess) return FS_ERR_CUDA;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusActive;
+  *ready = cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+  if (!*ready) cudaGetLastError();
+  return FS_OK;
 }
 
 // Samples per sub-block of the sums over nodes, or 0: a caller's position table (its
@@ -656,36 +667,41 @@ static int seg_node_sub(const fs_seg *seg) { return seg->eph ? 0 : node_sub(seg-
 static fs_status earth_table(fs_seg *seg, cudaStream_t st) {
   const unsigned nb = (unsigned)((seg->g.n + 255) / 256);
   const int sb = seg_node_sub(seg);
+  fs_status s;
   if (sb) {
-    if (!seg->nodes) {
+    if (!seg->nodes_ready) {
       NodeTab v;
-      const fs_status s = alloc_table(&seg->nodes, node_tab_view(seg->g, sb, nullptr, &v));
+      s = alloc_table(&seg->nodes, node_tab_view(seg->g, sb, nullptr, &v));
       if (s != FS_OK) return s;
       node_tab_view(seg->g, sb, (char *)seg->nodes, &v);
       const int64_t most = std::max<int64_t>(v.nn, kNodeSc);
       k_node_tables<<<(unsigned)((most + 63) / 64), 64, 0, st>>>(seg->g, v);
       seg->ctx->launches += 1;
-    }
-    if (!seg->xdf) {
-      const fs_status s = alloc_table((void **)&seg->xdf, sizeof(float2) * seg->g.n);
+      s = table_launched(st, &seg->nodes_ready);
       if (s != FS_OK) return s;
     }
+    s = alloc_table((void **)&seg->xdf, sizeof(float2) * seg->g.n);
+    if (s != FS_OK) return s;
     seg->ctx->launches += 1;
     return cuda_status(launch_pdl(k_data32, dim3(nb), dim3(256), 0, st, seg->g.n, seg->x64, seg->xdf));
   }
-  if (!seg->etab64) {
-    const fs_status s = alloc_table(&seg->etab64, sizeof(dbl4) * seg->g.n);
+  if (!seg->etab64_ready) {
+    s = alloc_table(&seg->etab64, sizeof(dbl4) * seg->g.n);
     if (s != FS_OK) return s;
     k_earth_table64<<<nb, 256, 0, st>>>(seg->g, (dbl4 *)seg->etab64);
     seg->ctx->launches += 1;
+    s = table_launched(st, &seg->etab64_ready);
+    if (s != FS_OK) return s;
   }
   if (!seg->eph) {
-    if (!seg->etab32) {
-      const fs_status s = alloc_table(&seg->etab32, etab32_bytes(seg->g.n));
+    if (!seg->etab32_ready) {
+      s = alloc_table(&seg->etab32, etab32_bytes(seg->g.n));
       if (s != FS_OK) return s;
       const unsigned nt = nb > 2 ? nb : 2;  // at least the 257 table entries
       k_earth_table32<<<nt, 256, 0, st>>>(seg->g.n, (const dbl4 *)seg->etab64, etab32_view(seg));
       seg->ctx->launches += 1;
+      s = table_launched(st, &seg->etab32_ready);
+      if (s != FS_OK) return s;
     }
     k_data32<<<nb, 256, 0, st>>>(seg->g.n, seg->x64, etab32_view(seg).X);
     seg->ctx->launches += 1;
