@@ -335,10 +335,9 @@ fs_status prepare_upsample(fs_seg *seg, const void *x_dev, cudaStream_t st, cons
 // the infinite line, whose kernel is (-c)^|k| / (2 sqrt 3) with c = 2 - sqrt 3: a causal
 // and an anticausal first-order recurrence,
 //   u_i = r_i - c u_{i-1},  v_i = r_i - c v_{i+1},  M_i = (u_i + v_i - r_i) / (2 sqrt 3).
-// A thread runs both over kSplS points after a warm-up of kSplK0 + kSplK1 steps (c^24 ~
-// 2e-14 of the data's scale is dropped); the first kSplK0, whose weight has fallen below
-// c^12 ~ 1e-7 by the strip, in FP32.  Five full steps per point, where a filter of 21 taps
-// in each direction took 42, in FP64, after 63 divisions per thread for the limit c.
+// A thread runs both over kSplS points after a warm-up of kSplK steps (c^24 ~ 2e-14 of the
+// data's scale is dropped).  Eight steps per point, where a filter of 21 taps in each
+// direction took 42, in FP64, after 63 divisions per thread for the limit c.
 //
 // That filter, kept up to now as the definition of the coefficients, stops at 21 terms:
 // with a = (-c)^21 its result is M_i (1 + a^2) - a (M_{i-21} + M_{i+21}).  The term in a
@@ -346,11 +345,12 @@ fs_status prepare_upsample(fs_seg *seg, const void *x_dev, cudaStream_t st, cons
 // of the same data stays the same to the last digits also where it is reported in FP64
 // (without it one coefficient in 2e4 moved by an FP32 ulp, F by up to 4e-9).
 //
-// FP32 segments run in double-floats, FP64 segments in double.  Latency bound (two chains
-// of 20 dependent steps per thread); kSplS = 8 keeps a 2-day series in 176 blocks.
-// Measured for 6 days at 2 s (516,984 points): 10.2 us in place of four kernels and 92 us.
+// FP32 segments run in double-floats, FP64 segments in double, the warm-up too.  Latency bound (two chains
+// of 32 dependent steps per thread); kSplS = 8 keeps a 2-day series in 176 blocks.
+// Measured for 6 days at 2 s (516,984 points): 11 us in place of four kernels and 92 us
+// (10.2 with the first 12 steps, whose weight is below c^12 ~ 1e-7, in FP32).
 constexpr int kSplEnd = 64;  // points at each end beyond which the Thomas factor c'_i is at its limit
-constexpr int kSplK0 = 12, kSplK1 = 12, kSplK = kSplK0 + kSplK1, kSplTap = 21, kSplS = 8, kSplThreads = 128;
+constexpr int kSplK = 24, kSplTap = 21, kSplS = 8, kSplThreads = 128;
 constexpr int kSplM = kSplThreads * kSplS;             // second derivatives a block computes
 constexpr int kSplTile = kSplM - 2 * kSplTap - 1;      // coefficients it writes
 constexpr double kSplC = 0.26794919243112270647, kSplG = 0.28867513459481288225;  // 2 - sqrt 3, 1/(2 sqrt 3)
@@ -437,16 +437,9 @@ __global__ void __launch_bounds__(kSplThreads) k_spline(const double *y, const f
   {
     const int j0 = threadIdx.x * kSplS;  // the strip's first point: l = j0, sr index j0 + kSplK
     const R c = n_from<R>(kSplC), gk = n_from<R>(kSplG);
-    constexpr float cf = (float)kSplC;
-    float uf = 0.f, vf = 0.f;
+    R u = zero, v = zero, us[kSplS], vs[kSplS];
 #pragma unroll
-    for (int k = 0; k < kSplK0; k++) {
-      uf = fmaf(-cf, uf, n_hi(sr[at8(j0 + k)]));
-      vf = fmaf(-cf, vf, n_hi(sr[at8(j0 + 2 * kSplK + kSplS - 1 - k)]));
-    }
-    R u = n_f32<R>(uf), v = n_f32<R>(vf), us[kSplS], vs[kSplS];
-#pragma unroll
-    for (int k = kSplK0; k < kSplK + kSplS; k++) {  // both chains side by side
+    for (int k = 0; k < kSplK + kSplS; k++) {  // both chains side by side
       u = n_sub(sr[at8(j0 + k)], n_mul(c, u));
       const R rb = sr[at8(j0 + 2 * kSplK + kSplS - 1 - k)];
       v = n_sub(rb, n_mul(c, v));
