@@ -308,16 +308,6 @@ cudaError_t fft64_twiddles(double2 *tw, int64_t n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Threads per block of a pass of `threads` threads: 128, or fewer when that leaves SMs
-// without a block: a small transform has to reach every SM's FP64 pipe (two transforms of
-// 2^16 points, 8192 threads in a radix-16 pass: 13.0 us in 64 blocks of 128, 11.9 us in 256
-// blocks of 32).
-static int block64(int64_t threads, int most) {
-  int b = most;
-  while (b > 32 && threads < (int64_t)b * 2 * 148) b >>= 1;
-  return b;
-}
-
 cudaError_t fft64(double2 *buf, double2 *tmp, const double2 *twiddle, int64_t n, int batch, int sign,
                   cudaStream_t st, int64_t *launches, double2 **out) {
   int lg = 0;
@@ -326,9 +316,8 @@ cudaError_t fft64(double2 *buf, double2 *tmp, const double2 *twiddle, int64_t n,
   double2 *dst = tmp;
   int log2p = 0;
   cudaError_t e = cudaSuccess;
-  auto pass = [&](void (*kern)(const double2 *, double2 *, const double2 *, int64_t, int, int, int), int lr, int most) {
+  auto pass = [&](void (*kern)(const double2 *, double2 *, const double2 *, int64_t, int, int, int), int lr, int nt) {
     const int64_t threads = (n >> lr) * batch;
-    const int nt = block64(threads, most);
     if (e == cudaSuccess)
       e = launch_pdl(kern, dim3((unsigned)((threads + nt - 1) / nt)), dim3(nt), 0, st, src, dst, twiddle, n, log2p,
                      sign, batch);
