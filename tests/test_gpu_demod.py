@@ -109,3 +109,24 @@ def test_short_sampling_intervals_match_oracle(fs, dt, n):
         a2, b2 = ab.cpu().numpy()
         for got, want in ((a2, ref.a2), (b2, ref.b2)):
             assert abs(got / want - 1) < 1e-6 + 4.8e-7 / np.sqrt(want)
+
+
+# Up to 16 sky positions, and two blocks of nodes per SM (4 positions of this series on 152
+# SMs), the node kernel sets the search up itself.
+@pytest.mark.parametrize("n,nfft,few,many", [(5000, 8192, 16, 17), (258492, 1 << 18, 4, 5), (258492, 1 << 18, 2, 17)])
+def test_set_up_in_the_node_kernel_changes_nothing(fs, n, nfft, few, many):
+    """The positions that two searches share have the same F and crossings, to the bit."""
+    dt, rng = 2.0, np.random.default_rng(n + many)
+    ctx = fs.Context(W.Detector(lambda_e0=1.0))
+    seg = fs.Segment(ctx, _dev(rng.standard_normal(n), torch.float32), dt, nfft, 435.1875, 2 * dt)
+    alpha, delta = _dev(rng.uniform(0, 2 * np.pi, many)), _dev(np.arcsin(rng.uniform(-1, 1, many)))
+    f1 = _dev([-1e-8, -3e-9, 0.0])
+    a = fs.search(ctx, seg, alpha[:few].contiguous(), delta[:few].contiguous(), f1, 14.0)
+    assert ctx.sync_status() == 0
+    Fa, ca = a.F.clone(), sorted(zip(*(v.tolist() for v in a.candidates())))
+    b = fs.search(ctx, seg, alpha, delta, f1, 14.0)
+    assert ctx.sync_status() == 0
+    assert torch.equal(b.F[:3 * few], Fa)
+    assert ca == sorted(c for c in zip(*(v.tolist() for v in b.candidates())) if c[0] < few)
+    again = fs.search(ctx, seg, alpha[:few].contiguous(), delta[:few].contiguous(), f1, 14.0)  # the counters are zero again
+    assert torch.equal(again.F, Fa)
