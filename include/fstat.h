@@ -300,14 +300,17 @@ typedef struct {
  * Eqs. OS and Fab over the segment's original samples (no resampling; phase
  * f0 (t + phi_m) + fl phi_m + f1 (t^2/2 + t phi_m), as in the fine search of
  * Sec. VI.C as run in Sec. VII): sums as double-floats with the orbital
- * phase in FP64 (FP64 throughout with a caller's position table).  F_dev: npt doubles.  grad_dev: NULL or [npt][4]
+ * phase in FP64, over a few nodes per block of samples (sampling intervals up
+ * to 16 s, 1024 samples or more) or over every sample (FP64 throughout, over
+ * every sample, with a caller's position table).  F_dev: npt doubles.  grad_dev: NULL or [npt][4]
  * doubles dF/d(f0, f1, alpha, delta).  hess_dev: NULL or [npt][10] doubles,
  * the upper triangle row by row of the Hessian of F.  metric_dev: NULL or [npt][10]
  * doubles, the upper triangle row by row of the reduced Fisher matrix
  * <m_i m_j> - <m_i><m_j> of the phase derivatives m_i = 2 pi dPhi/dtheta_i
  * (Eq. redFm-def, rad^2 per unit parameter^2).  The first call on a segment
- * builds an FP64 table of the orbital and sidereal angles (32 bytes per
- * sample, released with the segment). */
+ * builds tables of the orbital and sidereal angles at the nodes or samples (at
+ * most 72 bytes per sample, with the data as double-floats; released with the
+ * segment). */
 FS_API fs_status fs_fstat_points(fs_ctx *ctx, fs_seg *seg, const fs_point *pts_dev, int32_t npt,
                                  double *F_dev, double *grad_dev, double *hess_dev, double *metric_dev,
                                  void *stream);
@@ -317,8 +320,10 @@ FS_API fs_status fs_fstat_points(fs_ctx *ctx, fs_seg *seg, const fs_point *pts_d
  * times of Eq. eq:Bt, spline values, a and b at those times) with the phase
  * Psi_j = fl phi_m(t_j) + f1 (t_j^2/2 + t_j phi_m(t_j)) + f0 j dt, and F of Eq. OS.  At
  * f0 = k / (nfft dt) it is fs_search's F at bin k (the zero-padded DFT of
- * Eq. eq:DFT), between Fourier frequencies the same sum off the grid.  FP32 with
- * double-float phases, as fs_search.  F_dev: npt doubles.  Segments of
+ * Eq. eq:DFT) to about 2e-6 of it: the source times are solved sample by sample
+ * here (1e-9 s), from polynomials of the delay there (1e-12 s).  Between Fourier
+ * frequencies it is the same sum off the grid.  FP32 with double-float phases,
+ * as fs_search.  F_dev: npt doubles.  Segments of
  * precision FS_PREC_F32 with FS_INTERP_SPLINE2X and the analytic Earth only
  * (otherwise FS_ERR_UNSUPPORTED). */
 FS_API fs_status fs_fstat_resampled(fs_ctx *ctx, fs_seg *seg, const fs_point *pts_dev, int32_t npt,

@@ -111,10 +111,11 @@ __device__ __forceinline__ float df_mul_frac(df32 a, df32 b) {
 // so the order of a whole chain holds.  It does nothing in a kernel launched the ordinary
 // way.  Its pointers are not declared __restrict__: the data they point to may still change
 // when such a kernel starts, and the qualifier's promise that it does not would let a load
-// take the read-only path or move above the wait.  (Letting the next kernel start while blocks of the one before are still at work,
-// griddepcontrol.launch_dependents, measured no faster on a search of one template and
-// 40% slower on a segment load, whose waiting blocks then sit beside the working ones:
-// 148.6 us without, 209 us with it, 164 us with ordinary launches.)
+// take the read-only path or move above the wait.  (Letting the next kernel start while
+// blocks of the one before are still at work, griddepcontrol.launch_dependents, measured no
+// faster on a search of one template and 40% slower on a segment load, whose waiting blocks
+// then sit beside the working ones: 148.6 us without, 209 us with it, 164 us with ordinary
+// launches.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
@@ -162,7 +163,7 @@ struct SkyConst32 {
   float rcd, zsd;    // (r_e/c) cos(delta), (z/c) sin(delta)  [s]
   float ea[5];       // a = ea0 cos2x + ea1 sin2x + ea2 cos x + ea3 sin x + ea4, x = alpha - theta
   float eb[4];       // b = eb0 cos2x + eb1 sin2x + eb2 cos x + eb3 sin x
-  df32 ca2, sa2, rcd2, zsd2;  // ca, sa, rcd, zsd in two words (the demodulation's nodes)
+  df32 ca2, sa2, rcd2, zsd2;  // ca, sa, rcd, zsd in two words (the demodulation's nodes; unset elsewhere)
 };
 // FP64 counterpart.
 struct SkyConst64 {

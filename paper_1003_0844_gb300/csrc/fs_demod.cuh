@@ -1,7 +1,10 @@
-// One output sample of the FP32 resampling of Sec. VI.A (A1): the source time of
-// Eq. (eq:Bt), the data there, a and b, the delay and the spindown phase argument,
-// shared by the coarse search's demodulation (k_demod32) and the kernels of the
-// resampled F at continuous points (fs_adjoint.cu).
+// The FP32 resampling of Sec. VI.A (A1): what the coarse search's two forms of it share, and
+// one output sample of the form that solves Eq. (eq:Bt) for every sample (resample_sample:
+// the source time, the data there, a and b, the delay and the spindown phase argument).
+// That one serves k_demod32 (position tables, nearest neighbour, sampling intervals above
+// 16 s) and the kernels of the resampled F at continuous points (fs_adjoint.cu); the coarse
+// search with the analytic Earth takes the delay from polynomials (k_demod_poly), whose F
+// differs from the resampled one by the FP32 Newton step's 1e-9 s, 2e-6 of F.
 #pragma once
 #include "fs_common.cuh"
 
@@ -34,7 +37,7 @@ struct DemodArgs {
   float2 *partial;            // [nsky][gridDim.x]: block sums of a^2, b^2
   double *tsrc;               // optional [n] (first sky only)
   // demodulation by nodes (dem_block(dt) > 0): the segment's node tables and, per sky and
-  // block of 2^dlg samples, the polynomials of the delay, a and b (kDemCoef float4)
+  // block of nodes.K samples, the polynomials of the delay, a and b (kDemCoef float4)
   DemNodes nodes;
   float4 *dcoef;              // [nsky][nodes.nb][kDemCoef]
   // k_demod_nodes also finishes the sky: its norm from the blocks' sums (done: blocks

@@ -55,9 +55,10 @@ __host__ __device__ inline void sky_constants(double alpha, double delta, double
 }
 
 // The factors of the sky constants that depend on the detector alone, computed once per
-// context (by the device, so that they are the values its kernels would compute).  What is left per sky is two sine/cosine pairs: computing all
-// eighteen sines and cosines of sky_constants per sky took one thread 13 us, a third of
-// a single-template search of one day.
+// context (by the device, so that they are the values its kernels would compute).  What is
+// left per sky is two sine/cosine pairs: computing all eighteen sines and cosines of
+// sky_constants per sky took one thread 13 us, a third of a single-template search of one
+// day.
 struct DetConst {
   double ce, se;                  // obliquity
   double s2g, c2g, sl, cl, s2l, c2l;  // of 2 gamma, the latitude and twice the latitude
@@ -188,12 +189,12 @@ __device__ inline double source_time64(double tb, const SkyConst64 &K, const Seg
   const float p1 = delay32(tf - delay32(tf, K, g), K, g);
   const double t1 = tb - (double)p1;
   Geo64 q = geometry64(t1, K, g);
-  const double d = -(q.phi - (tb - t1)) / (1.0 + q.phidot), e = kOmegaR * d;  // tb - t1 is exact
+  const double d = -(q.phi - (tb - t1)) / (1.0 + q.phidot), e = kOmegaR * d;  // tb - t1: exact but for t1 near 0 (6e-14 s)
   q.dphi = q.phidot * d;  // kept beside phi: added to it, half a rounding of 500 s would be lost
   const double cx = fma(q.sx, e, q.cx);
   q.sx = fma(-q.cx, e, q.sx);
   q.cx = cx;
-  q.t1 = t1;  // exact: tb less an FP32 number
+  q.t1 = t1;  // rounded once; d is relative to the rounded value
   q.d = d;
   *geo = q;
   return t1 + d;

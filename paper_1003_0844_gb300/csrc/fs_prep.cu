@@ -345,7 +345,7 @@ fs_status prepare_upsample(fs_seg *seg, const void *x_dev, cudaStream_t st, cons
 // of the same data stays the same to the last digits also where it is reported in FP64
 // (without it one coefficient in 2e4 moved by an FP32 ulp, F by up to 4e-9).
 //
-// FP32 segments run in double-floats, FP64 segments in double, the warm-up too.  Latency bound (two chains
+// FP32 segments run in double-floats, FP64 segments in double.  Latency bound (two chains
 // of 32 dependent steps per thread); kSplS = 8 keeps a 2-day series in 176 blocks.
 // Measured for 6 days at 2 s (516,984 points): 11 us in place of four kernels and 92 us
 // (10.2 with the first 12 steps, whose weight is below c^12 ~ 1e-7, in FP32).

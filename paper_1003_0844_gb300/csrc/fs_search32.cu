@@ -2,11 +2,14 @@
 // the per-sky resampling/demodulation (A1) and the host orchestration of the
 // transform passes (device code in fs_pass32.cuh).
 //
-// Per sky (A1, k_demod32): source times t_j of Eq. (eq:Bt) by one Newton
-// step from a first delay estimate, the spline value x~_j (Sec. VI.A),
+// Per sky (A1): source times t_j of Eq. (eq:Bt), the spline value x~_j (Sec. VI.A),
 // a_j, b_j (Sec. II), the heterodyne factor exp(-2 pi i fl phi_m(t_j)) and
 // the spindown phase argument Q_j = t_j^2/2 + t_j phi_m(t_j) (Eq. phas) kept
-// as a double-float.  Output per sky: y^a_j, y^b_j (float2) and Q_j.
+// as a double-float.  The delay, a and b come from polynomials through a few nodes per
+// block of samples (k_demod_nodes, k_demod_poly); for a caller's position table, the
+// nearest-neighbour resampler and sampling intervals above 16 s every sample takes one
+// Newton step from a first delay estimate (k_demod32).  Output per sky: y^a_j, y^b_j
+// (float2) and Q_j.
 #include <stdio.h>
 #include <algorithm>
 #include "fs_demod.cuh"
@@ -345,8 +348,7 @@ __global__ void __launch_bounds__(128) k_demod_nodes(DemodArgs A, SetupArgs U) {
   const df32 cx = df_add(df_mul(K.ca2, ct), df_mul(K.sa2, sn)), sx = df_sub(df_mul(K.sa2, ct), df_mul(K.ca2, sn));
   constexpr float wo = (float)kOmegaO, wr = (float)kOmegaR;
   float ph = P.hi + fmaf(K.rcd, cx.hi, K.zsd);
-#pragma unroll
-  for (int it = 0; it < 1; it++) {
+  {
     const float eo = wo * ph, er = wr * ph, c1 = fmaf(-0.5f * er, er, 1.f), s1 = er - er * er * er * (1.f / 6.f);
     ph = fmaf(eo, R.hi, fmaf(-0.5f * eo * eo, P.hi, P.hi)) + fmaf(K.rcd, fmaf(cx.hi, c1, -sx.hi * s1), K.zsd);
   }
@@ -713,7 +715,7 @@ static void pass_args(const fs_seg *seg, const Cfg32 &c, const Ws32 &w, int nspi
   p1->yb = w.yb;
   p1->qq = w.qq;
   p1->sky_stride = w.stride;
-  p1->f1df = w.f1df;  // filled by f1_to_df32 before the launches
+  p1->f1df = w.f1df;  // filled by k_setup or k_demod_nodes<true> before the transform
   p1->nspin = nspin;
   p1->nspin_fd = make_fastdiv((uint32_t)nspin);
   p1->N2 = c.sh.N2;

@@ -1,7 +1,10 @@
-// Plain FP64 form of the search: every step in double, the analytic model (or
-// the caller's position table) evaluated directly at each source time, the spline in double, and the
-// zero-padded transform by the FP64 radix-2 Stockham FFT.  It is the
-// all-FP64 comparison for the FP32 path on the same GPU.
+// Plain FP64 form of the search: the analytic model in double at each source time (two FP32
+// evaluations bring the first estimate near it, source_time64) or the caller's position
+// table, the spline in double, and the zero-padded transform in double on chip
+// (k_fft64_cols, k_fft64_rows; 2^21 points by the radix-16 passes of fs_fft64.cu).  It is
+// the FP64 comparison for the FP32 path on the same GPU; against sums in 64-bit mantissas
+// (1500 to 258,492 samples) F is right to 2e-11 .. 8e-11, as with five FP64 evaluations per sample:
+// the FP64 phase of 2e5 cycles decides it.
 #include <type_traits>
 #include "fs_internal.h"
 #include "fs_model.cuh"
@@ -102,7 +105,7 @@ __global__ void __launch_bounds__(256) k_finalize64(const double *partial, int n
 // warp instruction per 16 clocks and SM) and, for one template, by the latency of a launch:
 // the two take the place of the chirp kernel, four radix-16 passes through global memory
 // and the F kernel.  Measured, a search of one template of 2^16: 63.6 us, 89.2 us before (57
-// of them in those six kernels); 157 -> 61 us for a drawn one of 2^15.
+// of them in those six kernels).
 constexpr int kDft64Seq = 4;  // sequences per block at least: two columns (rows) of both signals
 
 // exp(-2 pi i e / nfft) from the table of e < nfft/2, 0 <= e < nfft
