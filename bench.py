@@ -59,9 +59,10 @@ def metric_name(workload: str) -> str:
     return "F-stat templates/s (N=%d, 2^%d FFT, %s) on 1 GB300" % (wl.n, wl.nfft.bit_length() - 1, workload)
 
 
-REFINE_FLOP_PER_SAMPLE = 194.0   # FP32 flops per sample and point of a climb pass: the moments (52,
-                                 # their packed pairs left out) and the sums of F, gradient and
-                                 # Hessian over the nodes (142), from ncu's FADD/FFMA/FMUL counts
+REFINE_FLOP_PER_SAMPLE = 322.0   # FP32 flops per sample and point of a climb pass: the moments (52 by
+                                 # ncu's FADD/FFMA/FMUL counts, which leave packed pairs out, and 128
+                                 # in packed pairs, counted in the source) and the sums of F, gradient
+                                 # and Hessian over the nodes (142 by ncu)
                                  # (profiles/k_points_refine_2d.md)
 ADJOINT_FLOP_PER_SAMPLE = 424.0  # FP32 flops per output sample and point of the adjoint's backward
                                  # kernel (F and the 26 sums of its gradient), from ncu's FADD/FFMA/FMUL
@@ -761,7 +762,7 @@ def main_refine(args):
                      "frac": achieved / FP32_PEAK_TFLOPS, "traffic": None,
                      "peak_kind": "FP32 CUDA-core peak from unit counts and max clock (152 SM x 128 x 2 x 2070 MHz)",
                      "flop_convention": "%d FP32 flop per sample and point per pass (ncu opcode counts of the "
-                                        "kernels; the whole step's time)" % REFINE_FLOP_PER_SAMPLE},
+                                        "kernels, packed pairs from the source; the whole step's time)" % REFINE_FLOP_PER_SAMPLE},
         "gpu_launches": int(stats["launches"]),
         "clocks": ck,
         "F_gain": {"median": float(np.median(gain)), "max": float(np.max(gain))},

@@ -23,7 +23,7 @@
 // length.  Eight values per thread: 64 to 128 threads per sequence, two (1024, 512 points)
 // to sixteen (64 points) sequences per block, which gives 128 to 256 blocks at L = 2^17 and
 // 2^18.
-// Measured for 6 days at 2 s (N = 258,492, L = 2^18): 14.0 + 18.4 + 12.0 us, against
+// Measured for 6 days at 2 s (N = 258,492, L = 2^18): 14.5 + 27 + 12 us, against
 // 107 us for fifteen launches of the radix-16 form (kept for series below 2049 samples,
 // where it takes fewer and shorter passes, and above 2^20, which these kernels' two
 // factors of 1024 do not reach).
