@@ -137,8 +137,9 @@ FS_API void fs_destroy(fs_ctx *ctx);
  * (Sec. VI.A): time/ephemeris tables on the grid t_m = m dt (analytic Earth,
  * Eqs. pha4-pha5, Sec. V), the Fourier x2 upsampled series and its natural
  * cubic spline.  x_dev holds n samples of type desc->x_dtype.  The segment
- * keeps its own device copies (about 40 bytes per sample) and may be reused
- * by any number of fs_search calls.  Non-finite samples latch
+ * keeps its own device copies, tables and the upsampler's plan (170 to 220
+ * bytes per sample; with FS_PREC_F64 also 8 nfft bytes of twiddles) and may be
+ * reused by any number of fs_search calls.  Non-finite samples latch
  * FS_ERR_NONFINITE.  Release with fs_seg_destroy. */
 FS_API fs_status fs_prepare_segment(fs_ctx *ctx, fs_seg **seg, const fs_segment_desc *desc,
                              const void *x_dev, void *stream);
