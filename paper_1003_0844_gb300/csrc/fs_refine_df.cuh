@@ -238,8 +238,21 @@ __host__ __device__ __forceinline__ FastSample fast_sample(const FastConst &c, c
   return s;
 }
 
-// One sample's terms of F's and the gradient's accumulators (k_points_fg).  WT: the sums
-// without the data carry the weight s.wt.
+// First derivatives of a or b with alpha (from the Fourier coefficients e) and with delta
+// (from their derivatives ed, the constant term apart) as double-floats.
+__host__ __device__ __forceinline__ df32 ab_alpha(const df32 *e, const FastSample &s) {
+  return df_add(df_sub(df_scale(df_sub(df_mul(e[1], s.c2), df_mul(e[0], s.s2)), 2.f), df_mul(e[2], s.sx)),
+                df_mul(e[3], s.cx));
+}
+__host__ __device__ __forceinline__ df32 ab_delta(const float *ed, const FastSample &s) {
+  return df_add(df_add(df_mul_f(s.c2, ed[0]), df_mul_f(s.s2, ed[1])), df_add(df_mul_f(s.cx, ed[2]), df_mul_f(s.sx, ed[3])));
+}
+
+// One sample's terms of F's and the gradient's accumulators (k_points_fg).  WT (sums over
+// nodes, x = 1): the sums without the data carry the weight s.wt, and the derivatives of a
+// and b are double-floats: a few hundred nodes average FP32's rounding of them less than the
+// thousands of samples they stand for (the sky gradient's error 2e-8 of F, 4e-8 .. 1e-7
+// with FP32 derivatives, 4e-8 over every sample).
 template <bool WT = false>
 __host__ __device__ __forceinline__ void fg_sample(const FastConst &c, const FastSample &s, df32 *acc) {
   const df32 ua = df_mul(s.x, s.a), ub = df_mul(s.x, s.b);
@@ -261,6 +274,13 @@ __host__ __device__ __forceinline__ void fg_sample(const FastConst &c, const Fas
   const df32 dP[4] = {df_add(s.t, s.phi), s.tu, df_mul(w, phia), df_mul(w, phide)};
   const float da[4] = {0.f, 0.f, a_a, a_d}, db[4] = {0.f, 0.f, b_a, b_d};
   const float cpf = s.cp.hi, spf = s.sp.hi;
+  df32 da2[2], db2[2];
+  if constexpr (WT) {
+    da2[0] = ab_alpha(c.ea, s);
+    da2[1] = df_add(ab_delta(c.ea_d, s), df32{c.ea_d[4], 0.f});
+    db2[0] = ab_alpha(c.eb, s);
+    db2[1] = ab_delta(c.eb_d, s);
+  }
 #pragma unroll
   for (int i = 0; i < 4; i++) {
     // x (da_i - 2 pi i a dP_i) (cp - i sp)
@@ -271,21 +291,35 @@ __host__ __device__ __forceinline__ void fg_sample(const FastConst &c, const Fas
     acc[12 + 2 * i] = df_add(acc[12 + 2 * i], df_mul(rb, s.sp));
     acc[13 + 2 * i] = df_add(acc[13 + 2 * i], df_mul(rb, s.cp));
     if (i >= 2) {
-      const float qa = xf * da[i], qb = xf * db[i];
-      acc[4 + 2 * i] = df_add_f(acc[4 + 2 * i], qa * cpf);
-      acc[5 + 2 * i] = df_add_f(acc[5 + 2 * i], -qa * spf);
-      acc[12 + 2 * i] = df_add_f(acc[12 + 2 * i], qb * cpf);
-      acc[13 + 2 * i] = df_add_f(acc[13 + 2 * i], -qb * spf);
+      if constexpr (WT) {
+        acc[4 + 2 * i] = df_add(acc[4 + 2 * i], df_mul(da2[i - 2], s.cp));
+        acc[5 + 2 * i] = df_sub(acc[5 + 2 * i], df_mul(da2[i - 2], s.sp));
+        acc[12 + 2 * i] = df_add(acc[12 + 2 * i], df_mul(db2[i - 2], s.cp));
+        acc[13 + 2 * i] = df_sub(acc[13 + 2 * i], df_mul(db2[i - 2], s.sp));
+      } else {
+        const float qa = xf * da[i], qb = xf * db[i];
+        acc[4 + 2 * i] = df_add_f(acc[4 + 2 * i], qa * cpf);
+        acc[5 + 2 * i] = df_add_f(acc[5 + 2 * i], -qa * spf);
+        acc[12 + 2 * i] = df_add_f(acc[12 + 2 * i], qb * cpf);
+        acc[13 + 2 * i] = df_add_f(acc[13 + 2 * i], -qb * spf);
+      }
     }
   }
   const df32 wa = WT ? df_mul(s.wt, s.a) : s.a, wb = WT ? df_mul(s.wt, s.b) : s.b;
   acc[20] = df_add(acc[20], df_mul(wa, s.a));
   acc[21] = df_add(acc[21], df_mul(wb, s.b));
-  const float af = wa.hi, bf = wb.hi;
-  acc[22] = df_add_f(acc[22], af * a_a);
-  acc[23] = df_add_f(acc[23], af * a_d);
-  acc[24] = df_add_f(acc[24], bf * b_a);
-  acc[25] = df_add_f(acc[25], bf * b_d);
+  if constexpr (WT) {
+    acc[22] = df_add(acc[22], df_mul(wa, da2[0]));
+    acc[23] = df_add(acc[23], df_mul(wa, da2[1]));
+    acc[24] = df_add(acc[24], df_mul(wb, db2[0]));
+    acc[25] = df_add(acc[25], df_mul(wb, db2[1]));
+  } else {
+    const float af = wa.hi, bf = wb.hi;
+    acc[22] = df_add_f(acc[22], af * a_a);
+    acc[23] = df_add_f(acc[23], af * a_d);
+    acc[24] = df_add_f(acc[24], bf * b_a);
+    acc[25] = df_add_f(acc[25], bf * b_d);
+  }
 }
 
 // One sample's terms of the Hessian's accumulators (k_points_h).  Near a maximum the
@@ -300,15 +334,8 @@ __host__ __device__ __forceinline__ void hess_sample(const FastConst &c, const F
   constexpr int OB = SIG == 2 ? 20 : 0;  // offset of signal b's pairs
   const float cx = s.cx.hi, sx = s.sx.hi, c2 = s.c2.hi, s2 = s.s2.hi, xf = s.x.hi, af = s.a.hi, bf = s.b.hi;
   // first derivatives of a, b (double-float)
-  const df32 a_a = df_add(df_sub(df_scale(df_sub(df_mul(c.ea[1], s.c2), df_mul(c.ea[0], s.s2)), 2.f),
-                                 df_mul(c.ea[2], s.sx)), df_mul(c.ea[3], s.cx));
-  const df32 b_a = df_add(df_sub(df_scale(df_sub(df_mul(c.eb[1], s.c2), df_mul(c.eb[0], s.s2)), 2.f),
-                                 df_mul(c.eb[2], s.sx)), df_mul(c.eb[3], s.cx));
-  const df32 a_d = df_add(df_add(df_add(df_mul_f(s.c2, c.ea_d[0]), df_mul_f(s.s2, c.ea_d[1])),
-                                 df_add(df_mul_f(s.cx, c.ea_d[2]), df_mul_f(s.sx, c.ea_d[3]))),
-                          df32{c.ea_d[4], 0.f});
-  const df32 b_d = df_add(df_add(df_mul_f(s.c2, c.eb_d[0]), df_mul_f(s.s2, c.eb_d[1])),
-                          df_add(df_mul_f(s.cx, c.eb_d[2]), df_mul_f(s.sx, c.eb_d[3])));
+  const df32 a_a = ab_alpha(c.ea, s), b_a = ab_alpha(c.eb, s);
+  const df32 a_d = df_add(ab_delta(c.ea_d, s), df32{c.ea_d[4], 0.f}), b_d = ab_delta(c.eb_d, s);
   // second derivatives of a, b (FP32)
   const float a_aa = -4.f * c.eaf[0] * c2 - 4.f * c.eaf[1] * s2 - c.eaf[2] * cx - c.eaf[3] * sx;
   const float b_aa = -4.f * c.ebf[0] * c2 - 4.f * c.ebf[1] * s2 - c.ebf[2] * cx - c.ebf[3] * sx;
