@@ -59,10 +59,10 @@ def metric_name(workload: str) -> str:
     return "F-stat templates/s (N=%d, 2^%d FFT, %s) on 1 GB300" % (wl.n, wl.nfft.bit_length() - 1, workload)
 
 
-REFINE_FLOP_PER_SAMPLE = 322.0   # FP32 flops per sample and point of a climb pass: the moments (52 by
+REFINE_FLOP_PER_SAMPLE = 330.0   # FP32 flops per sample and point of a climb pass: the moments (52 by
                                  # ncu's FADD/FFMA/FMUL counts, which leave packed pairs out, and 128
                                  # in packed pairs, counted in the source) and the sums of F, gradient
-                                 # and Hessian over the nodes (142 by ncu)
+                                 # and Hessian over the nodes (151 by ncu)
                                  # (profiles/k_points_refine_2d.md)
 ADJOINT_FLOP_PER_SAMPLE = 424.0  # FP32 flops per output sample and point of the adjoint's backward
                                  # kernel (F and the 26 sums of its gradient), from ncu's FADD/FFMA/FMUL

@@ -27,13 +27,15 @@
 // by two 64-bit integer additions (units of 2^-64 cycles: reduction modulo 1 is free).
 //
 // Accuracy (19 lengths from 1024 samples to 6 days at 0.5 to 16 s, against sums in 64-bit
-// mantissas, worst of four points each): F 4e-14 .. 2e-11, the gradient 3e-14 .. 4e-11 and the
-// Hessian 1e-13 .. 1e-11 of F times the phase derivatives that meet in them; over every
+// mantissas, worst of four points each): F 4e-14 .. 2e-11, the gradient 1e-14 .. 4e-11 and the
+// Hessian 6e-14 .. 2e-11 of F times the phase derivatives that meet in them; over every
 // sample it is F 1e-11 .. 3e-10, gradient 4e-12 .. 3e-10, Hessian 2e-12 .. 1e-9, bound by the
 // FP64 phase of each sample (3e-11 cycles).  With blocks of 512 s whatever the length (one of
 // 256 samples for a series of 200) the gradient was off by up to 1e-8, the Hessian by 3e-7.
+// The sky gradient, whose parts cancel, ends at 2e-9 .. 5e-8 of F (3e-8 .. 2e-7 over every
+// sample, with FP32 derivatives of a and b).
 // Measured, 256 points of a 2-day series at 2 s with gradient and Hessian: 4.72 ms over every
-// sample, 0.27 ms this way, about half of it k_moments and half the sums over nodes.
+// sample, 0.28 ms this way, about half of it k_moments and half the sums over nodes.
 #pragma once
 
 namespace fs {
